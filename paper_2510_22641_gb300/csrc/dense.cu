@@ -114,13 +114,19 @@ void dense_plan(int M, int n_rt, int steps, int pairs, int* nt_out, int* split_o
   }
 }
 
+// p.apart (a batched verification's rows, at most kMaxMidRows, so nt <= 128 and two accumulators of 2 nt columns fit
+// TMEM): hi and lo products accumulate apart, as in the GEMV: one accumulator for both is cut off to its own last
+// bit twice per 16 columns instead of once.  13B verification, logits against 64 bits: 2.67e-5 with one
+// accumulator, 2.49e-5 with two, in the same time (27.2 ms for 16 requests' 24 tokens either way).
 // w: the site's weight maps; b: hi / lo maps of the rows' parts with p.nt / 2-row boxes (p.nt and p.split
 // from dense_plan).  Fills in the tile counts.
 cudaError_t dense_launch(Epi e, const CUtensorMap* w, const CUtensorMap* b, DenseParams p, int num_sms,
                          cudaStream_t s, bool pdl) {
   if (p.M < 1 || p.nt < 32 || p.nt > kDnMaxTok || p.nt % 32 || p.K % kTileK || p.n_rt < 1 || p.split < 1 ||
-      p.split > kDnMaxSplit || p.split * kTileK > p.K || (e == Epi::ARGMAX && p.M > kMaxMidRows))
+      p.split > kDnMaxSplit || p.split * kTileK > p.K || (e == Epi::ARGMAX && p.M > kMaxMidRows) ||
+      (p.apart && 2 * p.nt > kDnMaxTok))
     return cudaErrorInvalidValue;
+  p.lo_cols = p.apart ? p.nt : 0;
   p.tok_tiles = (p.M + p.nt - 1) / p.nt;
   p.stages = dense_stages(p.nt);
   const int ring = p.stages * (static_cast<int>(kWTileBytes) + p.nt * 128);

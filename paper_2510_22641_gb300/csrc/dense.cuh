@@ -77,6 +77,8 @@ struct DenseParams {
   int tok_tiles, nt;        // token tiles of nt tokens
   int split;                // CTA pairs that share one tile's reduction (the cluster holds `split` pairs)
   int stages;
+  int apart;                // 1: hi and lo products accumulate apart (nt <= 128)
+  int lo_cols;              // TMEM columns from a hi to a lo accumulator: nt with apart, 0 (the same one) without
   int seg_rows, seg_base;   // QKV: rows per source matrix, segment of the site's first matrix (0 q, 1 k, 2 v)
   float eps;
   DevState* st;             // error word, argmax keys; kv_len of one request
@@ -561,7 +563,7 @@ __global__ void __launch_bounds__(kDnThreads, 1)
   const uint32_t half_part = static_cast<uint32_t>(nt) * 64;  // bytes of this CTA's hi (or lo) rows of a stage
   const uint32_t stage_bytes = kWTileBytes + 2 * half_part;
   int tmem_cols = 32;
-  while (tmem_cols < 2 * nt) tmem_cols <<= 1;
+  while (tmem_cols < 2 * (nt + p.lo_cols)) tmem_cols <<= 1;
   const uint32_t acc_stride = static_cast<uint32_t>(tmem_cols) >> 1;
   uint8_t* ring = smem + S::kRing;
 
@@ -671,7 +673,7 @@ __global__ void __launch_bounds__(kDnThreads, 1)
           break;
         }
         tmem_fence_after();
-        const uint32_t d = tmem + static_cast<uint32_t>(b) * acc_stride;
+        const uint32_t d = tmem + static_cast<uint32_t>(b) * acc_stride, dl = d + static_cast<uint32_t>(p.lo_cols);
         for (int ks = 0; ks < k_steps; ++ks) {
           if (!dense_wait_warp(&full[s], ph, p.st)) {
             set_error(p.st, DERR_TIMEOUT);
@@ -680,13 +682,13 @@ __global__ void __launch_bounds__(kDnThreads, 1)
           }
           tmem_fence_after();
           const uint64_t so = static_cast<uint64_t>((s * stage_bytes) >> 4);  // descriptor units of the stage
-          const uint32_t more = ks > 0 ? 1u : 0u;
+          const uint32_t more = ks > 0 ? 1u : 0u, more_lo = p.lo_cols ? more : 1u;
           if (elect_one()) {
 #pragma unroll
             for (int kk = 0; kk < kTileK / 16; ++kk) {
               // +32 bytes (2 descriptor units) per 16-element K slice inside the swizzled row
               umma_f16_pair(d, w0 + so + 2 * kk, h0 + so + 2 * kk, idesc, kk > 0 ? 1u : more);
-              umma_f16_pair(d, w0 + so + 2 * kk, l0 + so + 2 * kk, idesc, 1u);
+              umma_f16_pair(dl, w0 + so + 2 * kk, l0 + so + 2 * kk, idesc, kk > 0 ? 1u : more_lo);
             }
             umma_commit_pair(&empty[s], both);  // both CTAs' stage s may be refilled once these MMAs have read it
             if (ks == k_steps - 1) umma_commit_pair(&tfull[b], both);  // accumulator b is complete in both CTAs
@@ -778,6 +780,15 @@ __global__ void __launch_bounds__(kDnThreads, 1)
       }
       tmem_fence_after();
       const uint32_t acc = tmem + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(b) * acc_stride;
+      auto load_chunk = [&](int col, float (&v)[kDnChunk]) {  // 16 tokens of this thread's weight row
+        tmem_ld16(acc + col, v);
+        if (p.lo_cols) {
+          float lo[kDnChunk];
+          tmem_ld16(acc + p.lo_cols + col, lo);
+#pragma unroll
+          for (int i = 0; i < kDnChunk; ++i) v[i] += lo[i];
+        }
+      };
       float* land = reinterpret_cast<float*>(ring);  // [chunk / split][pair][128][kDnLandLd], over the stage ring
       if (p.split > 1) {
         __syncwarp();
@@ -787,7 +798,7 @@ __global__ void __launch_bounds__(kDnThreads, 1)
           const int own = c % p.split;
           if (own == sp || (k++ & 1) != g || !have) continue;  // the two groups share the other pairs' chunks
           float v[kDnChunk];
-          tmem_ld16(acc + c * kDnChunk, v);
+          load_chunk(c * kDnChunk, v);
           const uint32_t dst = map_cluster(
               smem_u32(land + ((c / p.split * p.split + sp) * kTileN + row) * kDnLandLd), static_cast<uint32_t>(2 * own + rank));
 #pragma unroll
@@ -800,7 +811,7 @@ __global__ void __launch_bounds__(kDnThreads, 1)
         for (int c0 = cfirst; c0 < n_tok; c0 += cstep) {
           float v[kDnChunk], cur[kDnChunk];
           __syncwarp();
-          tmem_ld16(acc + c0, v);
+          load_chunk(c0, v);
           if (p.split > 1) {  // the pairs' shares in pair order
             const int base = c0 / kDnChunk / p.split * p.split;
             float sum[kDnChunk];

@@ -826,10 +826,12 @@ static void row_scales(ssd_ctx* c, DenseParams& p, bool from_split) {
 }
 
 // x += (*scale) * W v over M rows (x fp32, stride x_stride) from the parts of kind `part`; with next_gain
-// also writes the next normed projection's parts (x * next_gain) and the rows' sums of squares.
+// also writes the next normed projection's parts (x * next_gain) and the rows' sums of squares.  apart: see
+// dense_launch (here and below).
 static ssd_status dense_resid(ssd_ctx* c, int M, const Site& s, int part, float* x, int x_stride, const float* scale,
-                              const __nv_bfloat16* next_gain) {
+                              const __nv_bfloat16* next_gain, bool apart = false) {
   DenseParams p{};
+  p.apart = apart;
   p.base = x;
   p.base_stride = x_stride;
   p.dst = x;
@@ -846,8 +848,9 @@ static ssd_status dense_resid(ssd_ctx* c, int M, const Site& s, int part, float*
 }
 
 // The gated MLP's first half over M normed rows (parts PART_X, scales as row_scales): h's parts.
-static ssd_status dense_gate(ssd_ctx* c, int M, const Site& s, int act, bool from_split) {
+static ssd_status dense_gate(ssd_ctx* c, int M, const Site& s, int act, bool from_split, bool apart = false) {
   DenseParams p{};
+  p.apart = apart;
   row_scales(c, p, from_split);
   p.act = act;
   p.nx_hi = c->part_hi[PART_H];
@@ -1016,6 +1019,7 @@ static void set_batch_rows(ssd_ctx* c, GemvParams& p, int R) {
 }
 
 static void set_batch_rows(ssd_ctx* c, DenseParams& p, int R) {
+  p.apart = 1;
   p.batch_rows = R;
   p.req_st = c->req;
   p.req_kv = static_cast<long long>(c->req_kv);
@@ -1063,10 +1067,10 @@ static ssd_status enqueue_layer_batch(ssd_ctx* c, int l, float* x, int x_stride,
     a.xo_ld = c->qdim;
     CKS(attn_run(c, R, a, M / R));
     const bool last = l + 1 >= c->cfg.n_layers;
-    CKS(dense_resid(c, M, c->layers[l].o, PART_O, x, x_stride, resid_scale_of(c, l), c->ffn_norm[l]));
-    CKS(dense_gate(c, M, c->layers[l].gateup, 0, false));
+    CKS(dense_resid(c, M, c->layers[l].o, PART_O, x, x_stride, resid_scale_of(c, l), c->ffn_norm[l], true));
+    CKS(dense_gate(c, M, c->layers[l].gateup, 0, false, true));
     return dense_resid(c, M, c->layers[l].down, PART_H, x, x_stride, resid_scale_of(c, l),
-                       last ? c->final_norm : c->attn_norm[l + 1]);
+                       last ? c->final_norm : c->attn_norm[l + 1], true);
   }
   GemvParams p{};
   p.x = x;
@@ -2585,9 +2589,10 @@ ssd_status ssd_lm_head(ssd_ctx* c, const float* x, int rows, int32_t* tok, float
 static ssd_status profile_dense(ssd_ctx* c, Epi e, int which, int rows, const Site& s, const GemvParams& g) {
   const int part = which == 1 ? PART_O : which == 3 ? PART_H : PART_X;
   CKS(split(c, part, g.x, g.x_stride, s.K, g.gain, rows));
-  if (e == Epi::RESID) return dense_resid(c, rows, s, part, g.dst, g.dst_stride, g.scale, nullptr);
-  if (e == Epi::GATE_SILU) return dense_gate(c, rows, s, 0, true);
+  if (e == Epi::RESID) return dense_resid(c, rows, s, part, g.dst, g.dst_stride, g.scale, nullptr, true);
+  if (e == Epi::GATE_SILU) return dense_gate(c, rows, s, 0, true, true);
   DenseParams p{};
+  p.apart = 1;
   row_scales(c, p, true);
   p.q_out = g.q_out;
   p.q_stride = g.q_stride;
