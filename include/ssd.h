@@ -339,9 +339,11 @@ SSD_API ssd_status ssd_last_launch_count(ssd_ctx* ctx, int64_t* prefill_launches
  * tokens or eos) keeps its tokens; its rows ride along unused until every request
  * is done.  Every request's rows are computed independently of the other
  * requests', so its tokens and accept lengths are those of the same request
- * decoded alone; the batched prefill and, beyond 16 verification rows, the dense
- * projections sum in an order that depends on the number of rows in the pass, so
- * there they agree up to logits that tie within rounding.  The single-request calls (ssd_prefill .. ssd_verify)
+ * decoded alone, up to logits that tie within rounding: a single prompt's prefill and,
+ * beyond 16 verification rows, a batch's verification sum their products in an order
+ * that depends on the number of rows.  A batched prefill does not: a request's cache
+ * rows and first token are the same bits whichever requests are prefilled with it.
+ * The single-request calls (ssd_prefill .. ssd_verify)
  * and the batched calls share the cache: a prefill of one kind invalidates the
  * other kind's decode state. */
 

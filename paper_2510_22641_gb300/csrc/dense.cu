@@ -94,14 +94,16 @@ cudaError_t attr_e() {
 //  * sharing a tile's K steps among `split` pairs (only when every tile has a cluster of its own) costs two
 //    exchanges through distributed shared memory, about 3000, and divides K steps and epilogue: 4096 x
 //    11008 at 77 rows takes 24 us with split 3, 78 us without.
-void dense_plan(int M, int n_rt, int steps, int pairs, int* nt_out, int* split_out) {
+// max_split = 1 keeps a tile's K steps together at every M: then a row's sums do not depend on M (the tokens per
+// tile change which MMA column a row takes, not the order of its products).
+void dense_plan(int M, int n_rt, int steps, int pairs, int max_split, int* nt_out, int* split_out) {
   const int n_rp = (n_rt + 1) / 2;
   long long best = -1;
   for (int t = (M + kDnMaxTok - 1) / kDnMaxTok; t <= (M + 31) / 32; ++t) {
     const int nt = ((M + t - 1) / t + 31) / 32 * 32;
     const int tiles = n_rp * ((M + nt - 1) / nt);
     const long long step = 4 * nt + 16 > 350 ? 4 * nt + 16 : 350;
-    for (int split = 1; split <= kDnMaxSplit && split <= steps; ++split) {
+    for (int split = 1; split <= max_split && split <= steps; ++split) {
       if (split > 1 && tiles > g_max_clusters[split].load()) break;
       const long long waves = split > 1 ? 1 : (tiles + pairs - 1) / pairs;
       const long long cost = waves * ((steps + split - 1) / split * step + 1000) + 75ll * nt / split + (split > 1 ? 3000 : 0);

@@ -77,6 +77,7 @@ struct DenseParams {
   int tok_tiles, nt;        // token tiles of nt tokens
   int split;                // CTA pairs that share one tile's reduction (the cluster holds `split` pairs)
   int stages;
+  int whole;                // 1: a tile's K steps stay with one CTA pair, whatever M (dense_plan)
   int apart;                // 1: hi and lo products accumulate apart (nt <= 128)
   int lo_cols;              // TMEM columns from a hi to a lo accumulator: nt with apart, 0 (the same one) without
   int seg_rows, seg_base;   // QKV: rows per source matrix, segment of the site's first matrix (0 q, 1 k, 2 v)

@@ -47,7 +47,7 @@ cudaError_t prefill_attrs();
 cudaError_t prefill_attn_launch(int head_dim, const CUtensorMap* maps, __nv_bfloat16* o_hi, __nv_bfloat16* o_lo,
                                 int o_ld, const FaRequests& rq, int n, int n_heads, int s_pad, float scale,
                                 DevState* st, cudaStream_t s, bool pdl);
-void dense_plan(int M, int n_rt, int steps, int pairs, int* nt_out, int* split_out);
+void dense_plan(int M, int n_rt, int steps, int pairs, int max_split, int* nt_out, int* split_out);
 cudaError_t dense_launch(Epi e, const CUtensorMap* w, const CUtensorMap* b, DenseParams p, int num_sms,
                          cudaStream_t s, bool pdl);
 cudaError_t dense_attrs();
@@ -790,7 +790,7 @@ static ssd_status dense(ssd_ctx* c, Epi e, int M, const Site& s, int part, Dense
   p.seg_rows = s.seg_rows;
   p.eps = c->cfg.rms_eps;
   p.st = c->st;
-  dense_plan(M, s.n_rt, s.K / kTileK, c->num_sms / 2, &p.nt, &p.split);
+  dense_plan(M, s.n_rt, s.K / kTileK, c->num_sms / 2, p.whole ? 1 : kDnMaxSplit, &p.nt, &p.split);
   const auto key = std::make_tuple(part, s.K, p.nt / 2);
   auto it = c->part_maps.find(key);
   if (it == c->part_maps.end()) {
@@ -826,12 +826,10 @@ static void row_scales(ssd_ctx* c, DenseParams& p, bool from_split) {
 }
 
 // x += (*scale) * W v over M rows (x fp32, stride x_stride) from the parts of kind `part`; with next_gain
-// also writes the next normed projection's parts (x * next_gain) and the rows' sums of squares.  apart: see
-// dense_launch (here and below).
+// also writes the next normed projection's parts (x * next_gain) and the rows' sums of squares.  p (here and
+// below): how the products are summed (apart, whole), the rest is filled in.
 static ssd_status dense_resid(ssd_ctx* c, int M, const Site& s, int part, float* x, int x_stride, const float* scale,
-                              const __nv_bfloat16* next_gain, bool apart = false) {
-  DenseParams p{};
-  p.apart = apart;
+                              const __nv_bfloat16* next_gain, DenseParams p = {}) {
   p.base = x;
   p.base_stride = x_stride;
   p.dst = x;
@@ -848,9 +846,7 @@ static ssd_status dense_resid(ssd_ctx* c, int M, const Site& s, int part, float*
 }
 
 // The gated MLP's first half over M normed rows (parts PART_X, scales as row_scales): h's parts.
-static ssd_status dense_gate(ssd_ctx* c, int M, const Site& s, int act, bool from_split, bool apart = false) {
-  DenseParams p{};
-  p.apart = apart;
+static ssd_status dense_gate(ssd_ctx* c, int M, const Site& s, int act, bool from_split, DenseParams p = {}) {
   row_scales(c, p, from_split);
   p.act = act;
   p.nx_hi = c->part_hi[PART_H];
@@ -860,14 +856,17 @@ static ssd_status dense_gate(ssd_ctx* c, int M, const Site& s, int act, bool fro
 }
 
 // All layers over the M input rows in x_pre through the dense projections: one request's P rows (row_map
-// null: row m at position m) or several requests' (row_map).  rq: the requests' rows for the attention.
+// null: row m at position m) or several requests' (row_map), whose projections do not share K steps, so that a
+// request's rows do not depend on the requests beside it.  rq: the requests' rows for the attention.
 static ssd_status enqueue_dense_layers(ssd_ctx* c, int M, const int4* row_map, const FaRequests& rq, int n_req) {
   const int dp = c->dp, L = c->cfg.n_layers;
   __nv_bfloat16 *qh = c->fa_parts, *ql = qh + c->fa_q_elems, *kh = qh + 2 * c->fa_q_elems, *kl = kh + c->fa_kv_elems,
                 *vh = kh + 2 * c->fa_kv_elems, *vl = kh + 3 * c->fa_kv_elems;
+  DenseParams sums{};
+  sums.whole = row_map != nullptr;
   // q/k/v of block l from the parts of kind `part`: K/V into the cache and, with attn, the attention's operands
   auto qkv = [&](int l, int part, bool from_split, bool attn) -> ssd_status {
-    DenseParams p{};
+    DenseParams p = sums;
     row_scales(c, p, from_split);
     p.abs_pos = 1;
     p.row_map = row_map;
@@ -903,10 +902,10 @@ static ssd_status enqueue_dense_layers(ssd_ctx* c, int M, const int4* row_map, c
     CK(prefill_attn_launch(c->cfg.head_dim, c->fa_maps, c->part_hi[PART_O], c->part_lo[PART_O], c->qdim, rq, n_req,
                            c->cfg.n_heads, c->fa_spad, 1.0f / sqrtf(static_cast<float>(c->cfg.head_dim)), c->st, c->cs,
                            c->use_pdl));
-    CKS(dense_resid(c, M, c->layers[l].o, PART_O, c->x_pre, dp, resid_scale_of(c, l), c->ffn_norm[l]));
-    CKS(dense_gate(c, M, c->layers[l].gateup, 0, false));
+    CKS(dense_resid(c, M, c->layers[l].o, PART_O, c->x_pre, dp, resid_scale_of(c, l), c->ffn_norm[l], sums));
+    CKS(dense_gate(c, M, c->layers[l].gateup, 0, false, sums));
     CKS(dense_resid(c, M, c->layers[l].down, PART_H, c->x_pre, dp, resid_scale_of(c, l),
-                    l + 1 < L ? c->attn_norm[l + 1] : nullptr));
+                    l + 1 < L ? c->attn_norm[l + 1] : nullptr, sums));
   }
   if (c->cfg.draft_exit_k == L && c->cfg.in_kind == SSD_IN_BLOCK) CKS(block_kv());
   return SSD_OK;
@@ -1067,10 +1066,12 @@ static ssd_status enqueue_layer_batch(ssd_ctx* c, int l, float* x, int x_stride,
     a.xo_ld = c->qdim;
     CKS(attn_run(c, R, a, M / R));
     const bool last = l + 1 >= c->cfg.n_layers;
-    CKS(dense_resid(c, M, c->layers[l].o, PART_O, x, x_stride, resid_scale_of(c, l), c->ffn_norm[l], true));
-    CKS(dense_gate(c, M, c->layers[l].gateup, 0, false, true));
+    DenseParams sums{};
+    sums.apart = 1;
+    CKS(dense_resid(c, M, c->layers[l].o, PART_O, x, x_stride, resid_scale_of(c, l), c->ffn_norm[l], sums));
+    CKS(dense_gate(c, M, c->layers[l].gateup, 0, false, sums));
     return dense_resid(c, M, c->layers[l].down, PART_H, x, x_stride, resid_scale_of(c, l),
-                       last ? c->final_norm : c->attn_norm[l + 1], true);
+                       last ? c->final_norm : c->attn_norm[l + 1], sums);
   }
   GemvParams p{};
   p.x = x;
@@ -2589,10 +2590,10 @@ ssd_status ssd_lm_head(ssd_ctx* c, const float* x, int rows, int32_t* tok, float
 static ssd_status profile_dense(ssd_ctx* c, Epi e, int which, int rows, const Site& s, const GemvParams& g) {
   const int part = which == 1 ? PART_O : which == 3 ? PART_H : PART_X;
   CKS(split(c, part, g.x, g.x_stride, s.K, g.gain, rows));
-  if (e == Epi::RESID) return dense_resid(c, rows, s, part, g.dst, g.dst_stride, g.scale, nullptr, true);
-  if (e == Epi::GATE_SILU) return dense_gate(c, rows, s, 0, true, true);
   DenseParams p{};
   p.apart = 1;
+  if (e == Epi::RESID) return dense_resid(c, rows, s, part, g.dst, g.dst_stride, g.scale, nullptr, p);
+  if (e == Epi::GATE_SILU) return dense_gate(c, rows, s, 0, true, p);
   row_scales(c, p, true);
   p.q_out = g.q_out;
   p.q_stride = g.q_stride;
