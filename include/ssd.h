@@ -118,7 +118,10 @@ typedef struct {
   int options;       /* SSD_OPT_* bits, 0 = the default path */
   int max_batch;     /* requests one batched decode may carry (0 or 1: single requests only; at most
                       * SSD_MAX_ROWS, with max_batch * (gamma_max + 1) <= 128; SSD_ARCH_LLAMA with
-                      * SSD_IN_IDENTITY or SSD_IN_MLP2).  The KV cache holds max_batch request slots. */
+                      * SSD_IN_IDENTITY or SSD_IN_MLP2).  The KV cache holds max_batch request slots, and
+                      * the batched prefill buffers for the rows of one pass: min(max_batch * max_seq, 8192)
+                      * rows of about 8 d_model + 16 n_heads head_dim + 4 d_ff bytes, or one prompt's
+                      * (max_seq rows) if that allocation fails.  SSD_OPT_PREFILL_ROWS takes neither. */
 } ssd_config;
 
 /* Extra weights of SSD_ARCH_T5, device bf16, [out][in], borrowed.  The
@@ -436,7 +439,7 @@ SSD_API ssd_status ssd_profile_projection(ssd_ctx* ctx, int which, int layer, in
 /* ---- Failure-path diagnostics (for tests of callers' error handling; no GPU fault is made) ---- */
 
 /* Host-side fault injection: after this call, the countdown-th device allocation
- * (kind SSD_FAULT_ALLOC: reported as SSD_ERR_OOM) or the countdown-th kernel launch
+ * (kind SSD_FAULT_ALLOC: reported as SSD_ERR_OOM, but see max_batch) or the countdown-th kernel launch
  * through the library's launch wrappers (kind SSD_FAULT_LAUNCH: reported as
  * SSD_ERR_CUDA, the kernel is not launched) of any ctx fails once, without
  * reaching the GPU.  kind SSD_FAULT_NONE or countdown <= 0 disarms.  Process-wide;

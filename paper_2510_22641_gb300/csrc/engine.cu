@@ -1573,6 +1573,7 @@ static ssd_status alloc(ssd_ctx* c, void** p, size_t bytes, bool clear = true) {
   cudaError_t e = injected_fault(SSD_FAULT_ALLOC) ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
   if (e != cudaSuccess) {
     *p = nullptr;
+    cudaGetLastError();  // a caller may go on with less: the next launch check must not see it
     return fail(c, SSD_ERR_OOM, "cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));
   }
   if (!clear) return SSD_OK;
@@ -1890,31 +1891,40 @@ static ssd_status create_impl(ssd_ctx* c, const ssd_config* cfg, const ssd_weigh
   CKS(alloc(c, reinterpret_cast<void**>(&c->in_vis), sizeof(__nv_bfloat16) * in_rows * d));
   {
     // row buffers of the dense projections: a prompt's (or the encoder's) rows, a batch's verification rows, or
-    // several prompts of a batch, up to kBatchPrefillRows (about there the projections run at the tensor rate).
-    // Written before they are read, so not cleared.
+    // several prompts of a batch, up to kBatchPrefillRows (about there the projections run at the tensor rate) or,
+    // where memory does not reach that far, one prompt.  A prefill through the decode kernels needs none of its
+    // own.  Written before they are read, so not cleared.
+    const bool fa = !t5 && !c->prefill_rows;  // with the prefill attention's operand parts
     const int S16 = (std::max(k.max_seq, c->max_enc) + kDnChunk - 1) / kDnChunk * kDnChunk;
-    c->part_rows = std::max(R, max_batch > 1 ? std::max(S16, std::min(max_batch * S16, kBatchPrefillRows)) : S16);
+    const int64_t many = std::max<int64_t>(S16, std::min<int64_t>(static_cast<int64_t>(max_batch) * S16, kBatchPrefillRows));
+    const int least = c->prefill_rows ? R : std::max(R, S16);
+    c->part_rows = c->prefill_rows ? R : std::max(R, max_batch > 1 ? static_cast<int>(many) : S16);
     c->part_ssq_ld = 4 * ((k.d_model + kTileN - 1) / kTileN);  // per 32 columns of x, whole 128-column tiles
     const size_t widths[3] = {d, static_cast<size_t>(qdim), std::max(static_cast<size_t>(k.d_ff), d)};
-    if (!t5) {  // the prefill attention's operand parts (K / V^T rows of each request padded to whole key blocks)
-      c->fa_spad = (c->part_rows + (max_batch > 1 ? max_batch * (kFaKRows - kDnChunk) : 0) + kFaKRows - 1) / kFaKRows * kFaKRows;
-      c->fa_q_elems = static_cast<size_t>(c->part_rows) * static_cast<size_t>(qdim);
-      c->fa_kv_elems = static_cast<size_t>(k.n_heads) * c->fa_spad * k.head_dim;
-    }
     // one allocation for all of them, cut at 1 KB boundaries (each allocation costs about 0.1 ms)
-    size_t bytes = 0;
-    auto carve = [&](size_t n) {
-      const size_t at = bytes;
-      bytes += (n + 1023) / 1024 * 1024;
-      return at;
-    };
-    const size_t rows = c->part_rows;
-    const size_t x_at = carve(sizeof(float) * rows * c->dp), rs_at = carve(sizeof(float) * rows),
-                 ssq_at = carve(sizeof(float) * rows * c->part_ssq_ld);
-    size_t part_at[6];
-    for (int i = 0; i < 6; ++i) part_at[i] = carve(sizeof(__nv_bfloat16) * rows * widths[i >> 1]);
-    const size_t fa_at = carve(sizeof(__nv_bfloat16) * (2 * c->fa_q_elems + 4 * c->fa_kv_elems));
-    CKS(alloc(c, reinterpret_cast<void**>(&c->part_mem), bytes, false));
+    size_t x_at, rs_at, ssq_at, part_at[6], fa_at, rows;
+    for (;; c->part_rows = least) {
+      rows = c->part_rows;
+      if (fa) {  // K / V^T rows of each request padded to whole key blocks
+        c->fa_spad = (c->part_rows + (max_batch > 1 ? max_batch * (kFaKRows - kDnChunk) : 0) + kFaKRows - 1) / kFaKRows * kFaKRows;
+        c->fa_q_elems = rows * static_cast<size_t>(qdim);
+        c->fa_kv_elems = static_cast<size_t>(k.n_heads) * c->fa_spad * k.head_dim;
+      }
+      size_t bytes = 0;
+      auto carve = [&](size_t n) {
+        const size_t at = bytes;
+        bytes += (n + 1023) / 1024 * 1024;
+        return at;
+      };
+      x_at = carve(sizeof(float) * rows * c->dp);
+      rs_at = carve(sizeof(float) * rows);
+      ssq_at = carve(sizeof(float) * rows * c->part_ssq_ld);
+      for (int i = 0; i < 6; ++i) part_at[i] = carve(sizeof(__nv_bfloat16) * rows * widths[i >> 1]);
+      fa_at = carve(sizeof(__nv_bfloat16) * (2 * c->fa_q_elems + 4 * c->fa_kv_elems));
+      const ssd_status r = alloc(c, reinterpret_cast<void**>(&c->part_mem), bytes, false);
+      if (r == SSD_OK) break;
+      if (r != SSD_ERR_OOM || c->part_rows <= least) return r;
+    }
     c->x_pre = reinterpret_cast<float*>(c->part_mem + x_at);
     c->part_rs = reinterpret_cast<float*>(c->part_mem + rs_at);
     c->part_ssq = reinterpret_cast<float*>(c->part_mem + ssq_at);
@@ -1923,7 +1933,7 @@ static ssd_status create_impl(ssd_ctx* c, const ssd_config* cfg, const ssd_weigh
       c->part_lo[i] = reinterpret_cast<__nv_bfloat16*>(c->part_mem + part_at[2 * i + 1]);
     }
     if (max_batch > 1) CKS(alloc(c, reinterpret_cast<void**>(&c->row_map), sizeof(int4) * c->part_rows));
-    if (!t5) {
+    if (fa) {
       const int H = k.n_heads, Dh = k.head_dim;
       c->fa_parts = reinterpret_cast<__nv_bfloat16*>(c->part_mem + fa_at);
       __nv_bfloat16* base = c->fa_parts;
