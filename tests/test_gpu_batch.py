@@ -5,7 +5,8 @@ Every request must match the oracle run on it alone (tokens up to an excused nea
 and draft logits at the stated tolerance, per-step accept lengths and kv_len bit-exact); the
 oracle's lockstep batch loop is pinned on the CPU to give each request exactly that run.
 Verification rows beyond 16 (4 requests at gamma >= 4, 16 requests at gamma = 6) go through the
-medium-M tensor-core kernel; fewer rows through the weight-streaming GEMV.
+dense projections; fewer rows of this tiny model through the small-matrix kernel (the LM head through
+the weight-streaming kernel).  test_gpu_batch_wide.py holds a model whose rows all stream.
 """
 import numpy as np
 import pytest
@@ -108,8 +109,8 @@ def check_request(r, ref, gamma):
 
 @pytest.mark.parametrize("s,gamma", [(0.05, 4), (0.2, 4), (1.0, 2), (0.05, 7), (0.2, 1)])
 def test_batch_ssd_matches_oracle_per_request(model4, tiny_bits, s, gamma):
-    """4 ragged requests; gamma = 4 and 7 verify 20 and 32 rows (medium-M kernel), gamma <= 2 at
-    most 12 (GEMV)."""
+    """4 ragged requests; gamma = 4 and 7 verify 20 and 32 rows (dense projections), gamma <= 2 at
+    most 12."""
     bw = tiny_batch(s=s)
     set_scale(model4, bw.base)
     got = gpu_batch(model4, bw, gamma)
@@ -144,8 +145,8 @@ def test_batch_ssd_equals_batch_greedy(model4, gamma):
 
 
 def test_batch_of_16_verifies_112_rows(tiny_bits):
-    """16 requests at gamma = 6: every verification projection carries 112 rows (7 chunks of the
-    medium-M kernel) and every drafting projection 16 rows."""
+    """16 requests at gamma = 6: every verification projection carries 112 rows (7 chunks of a
+    dense epilogue) and every drafting projection 16 rows."""
     bw = tiny_batch(batch=16, s=0.05, gamma=6)
     model, _, _ = make_model(bw.base, tiny_bits, gamma_max=6, max_seq=bw.max_seq(), max_batch=16)
     try:

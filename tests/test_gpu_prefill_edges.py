@@ -1,7 +1,7 @@
 """Prefill lengths around the tile edges of the prefill kernels, against the fp64 oracle.
 
-The prefill GEMM has 128-row tiles and the tensor-core attention 128-query blocks of 64-key steps,
-so lengths 1, 63..65, 127..129 and 200 hit an empty-but-one tile, partial key blocks, exact block
+The dense projections have tiles of 32 to 256 rows and the attention 128-query blocks of 64-key steps,
+so lengths 1, 63..65, 127..129 and 200 hit tiles with one row, partial key blocks, exact block
 ends and a ragged second query block, for head_dim 64 and 128.  A prompt of a single id with no
 visual rows is the smallest input.  Checked per length: every layer's K/V rows and the first
 token's logits.

@@ -1,12 +1,13 @@
 """Encoder-decoder (BLIP-2 FlanT5-shaped) CUDA path vs the fp64 encoder-decoder oracle, through the C ABI.
 
 Tiny workload: 2 encoder + 4 decoder layers, d=256, 4 heads x 64, V=2048.  The encoder runs through
-the tensor-core prefill GEMM (one 128-row tile for the default 48 encoder rows); a long case (130
-encoder rows, 150 new tokens) spans two row tiles (the second holds 2 rows), three 64-key attention
-chunks on both the encoder and the decoder side, and relative offsets beyond max_distance / 2 in
-both bucket schemes.  The row prefill (the decode kernels in 8-row chunks) is checked against the
-tensor-core one and the oracle, and a model with max_enc = 64 runs the cross-attention folded into
-the cross-q projection's epilogue (the fixture's max_enc = 160 keeps the separate kernel).  The
+the dense projections; a long case (130 encoder rows, 150 new tokens) spans several token tiles and
+17 blocks of encoder rows (the last holds 2), three 64-key attention chunks on both the encoder and
+the decoder side, and relative offsets beyond max_distance / 2 in both bucket schemes.  The row
+prefill (the decode kernels in 8-row chunks) is checked against the dense one and the oracle.  The
+tiny decoder's projections all run through the small-matrix kernel, with the cross-attention as a
+launch of its own; a wide model (d = 4160: too long for that kernel) with at most 128 encoder rows
+runs it folded into the cross-q projection's epilogue.  The
 FlanT5-xl-shaped case (24 + 24 layers, d=2048, V=32128) compares the oracle's prefill and first SSD
 steps with the GPU's and checks SSD == greedy over all 30 tokens.
 """
@@ -109,7 +110,7 @@ def test_t5_ssd_matches_oracle_and_gpu_greedy(tiny_model, tiny_bits, s, gamma):
 
 
 def test_t5_tensor_core_prefill_matches_row_prefill(tiny_model, tiny_bits):
-    """The encoder through the tcgen05 prefill GEMM and through the decode kernels in 8-row chunks
+    """The encoder through the dense projections and through the decode kernels in 8-row chunks
     give the same greedy stream within the oracle's tolerance; both match the oracle."""
     w = tiny(s=0.3, n_query=100, n_prompt=30, max_new=40)
     set_s(tiny_model, w)
@@ -130,28 +131,36 @@ def test_t5_tensor_core_prefill_matches_row_prefill(tiny_model, tiny_bits):
         assert_logits_close(logits[t], rlogits[t], f"tensor-core vs row prefill, logits of token {t}")
 
 
-@pytest.mark.parametrize("s,gamma", [(0.05, 4), (0.3, 3)])
-def test_t5_folded_cross_attention(tiny_model, tiny_bits, s, gamma):
-    """With max_enc <= 128 the cross-attention runs in the cross-q projection's epilogue: greedy and
-    SSD against the oracle, SSD == greedy bitwise, logits within tolerance of the separate
-    cross-attention kernel's (the fixture's max_enc = 160 keeps that path)."""
-    w = tiny(s=s)
-    fold, _, _ = make_t5_model(w, tiny_bits, gamma_max=GAMMA_MAX, max_seq=200, max_enc=64)
-    try:
-        set_s(fold, w)
-        gtoks, glogits, gst = gpu_decode(fold, w, 0)
-        toks, logits, st = gpu_decode(fold, w, gamma)
-    finally:
-        fold.close()
-    assert check(gtoks, glogits, gst, oracle_run(w, tiny_bits, 0), 0) >= 8
-    check(toks, logits, st, oracle_run(w, tiny_bits, gamma), gamma)
-    assert toks == gtoks
-    np.testing.assert_array_equal(logits, glogits)
-    set_s(tiny_model, w)
-    ktoks, klogits, _ = gpu_decode(tiny_model, w, 0)
-    n = common_prefix(gtoks, ktoks, klogits)
-    for t in range(min(n + 1, w.max_new)):
-        assert_logits_close(glogits[t], klogits[t], f"folded vs separate cross-attention, logits of token {t}")
+@pytest.mark.parametrize("head_dim", [64, 128])
+def test_t5_folded_cross_attention(head_dim):
+    """With max_enc <= 128 and a cross q beyond the small-matrix kernel (K = 4160) the cross-attention runs in the
+    cross-q projection's epilogue, 7 launches per decoder layer; with max_enc = 160 a launch of its own follows, 8
+    per layer.  Both against the oracle and each other, SSD == greedy bitwise at 2 to 16 rows.  Self q/k/v of this
+    width run through the weight-streaming kernel without rotation."""
+    shape = synth.T5Shape(n_enc=1, n_dec=2, d_model=4160, n_heads=384 // head_dim, head_dim=head_dim, d_ff=128, vocab=500)
+    w = tiny(shape=shape, draft_exit_k=1, in_hidden=128, n_query=20, n_prompt=11, max_new=18, s=0.3)
+    bits = synth.make_t5_weights(w)
+    ref = oracle_run(w, bits, 0)
+    out = {}
+    for max_enc, per_layer in ((64, 7), (160, 8)):
+        model, _, _ = make_t5_model(w, bits, gamma_max=15, max_seq=64, max_enc=max_enc)
+        try:
+            set_s(model, w)
+            toks, logits, st = gpu_decode(model, w, 0)
+            assert check(toks, logits, st, ref, 0) >= 8
+            # embed, layers, head, accept per step; setup, loop begin and copy-out around them
+            assert model.launch_counts()[1] == 3 + st["steps"] * (3 + per_layer * shape.n_dec)
+            for gamma in (1, 4, 8, 15):
+                t, lg, _ = gpu_decode(model, w, gamma)
+                assert t == toks, gamma
+                np.testing.assert_array_equal(lg, logits)
+            out[max_enc] = logits
+            model.set_logits_capture(None)
+        finally:
+            model.close()
+    # fp32 both, sums in another order: 1e-4 of the rms is ten times what two bf16 parts per activation leave
+    rms = float(np.sqrt(np.mean(out[160] ** 2)))
+    assert np.abs(out[64] - out[160]).max() <= 1e-4 * max(rms, np.abs(out[160]).max())
 
 
 def test_t5_long_encoder_and_decoder(tiny_model, tiny_bits):
