@@ -1,5 +1,6 @@
 // Launchers of the dense projections (ssd_dense_kernel) and of the operand split.
 #include <atomic>
+#include <initializer_list>
 
 #include "dense.cuh"
 
@@ -75,12 +76,15 @@ cudaError_t launch_e(const CUtensorMap* w, const CUtensorMap* b, const DensePara
   at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, ssd_dense_kernel<EPI>, w[0], w[1], w[2], b[0], b[1], p);
+  return cudaLaunchKernelEx(&cfg, p.apart ? ssd_dense_kernel<EPI, true> : ssd_dense_kernel<EPI, false>, w[0], w[1], w[2],
+                            b[0], b[1], p);
 }
 
 template <Epi EPI>
 cudaError_t attr_e() {
-  return cudaFuncSetAttribute(ssd_dense_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, DnSmem::kMax);
+  for (auto* k : {ssd_dense_kernel<EPI, false>, ssd_dense_kernel<EPI, true>})
+    if (cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, DnSmem::kMax)) return e;
+  return cudaSuccess;
 }
 
 }  // namespace
@@ -128,7 +132,6 @@ cudaError_t dense_launch(Epi e, const CUtensorMap* w, const CUtensorMap* b, Dens
       p.split > kDnMaxSplit || p.split * kTileK > p.K || (e == Epi::ARGMAX && p.M > kMaxMidRows) ||
       (p.apart && 2 * p.nt > kDnMaxTok))
     return cudaErrorInvalidValue;
-  p.lo_cols = p.apart ? p.nt : 0;
   p.tok_tiles = (p.M + p.nt - 1) / p.nt;
   p.stages = dense_stages(p.nt);
   const int ring = p.stages * (static_cast<int>(kWTileBytes) + p.nt * 128);
@@ -163,7 +166,7 @@ cudaError_t dense_attrs() {
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int n = 0;
-    if ((e = cudaOccupancyMaxActiveClusters(&n, ssd_dense_kernel<Epi::RESID>, &cfg))) return e;
+    if ((e = cudaOccupancyMaxActiveClusters(&n, ssd_dense_kernel<Epi::RESID, false>, &cfg))) return e;
     g_max_clusters[split].store(n);
   }
   return cudaSuccess;

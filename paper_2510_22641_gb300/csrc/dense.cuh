@@ -79,7 +79,6 @@ struct DenseParams {
   int stages;
   int whole;                // 1: a tile's K steps stay with one CTA pair, whatever M (dense_plan)
   int apart;                // 1: hi and lo products accumulate apart (nt <= 128)
-  int lo_cols;              // TMEM columns from a hi to a lo accumulator: nt with apart, 0 (the same one) without
   int seg_rows, seg_base;   // QKV: rows per source matrix, segment of the site's first matrix (0 q, 1 k, 2 v)
   float eps;
   DevState* st;             // error word, argmax keys; kv_len of one request
@@ -540,7 +539,8 @@ __device__ __forceinline__ void dense_chunk(const DenseParams& p, int rt, int m0
 // the s-th part of the K steps.  The pairs' accumulators meet through distributed shared memory: 16-token
 // chunk c belongs to pair c mod split, the others store their chunk into its (by then idle) stage ring, and
 // the owner adds them in pair order and runs the chunk's epilogue.
-template <Epi EPI>
+// APART: hi and lo products accumulate apart, the lo accumulator nt columns after the hi one (dense_launch).
+template <Epi EPI, bool APART>
 __global__ void __launch_bounds__(kDnThreads, 1)
     ssd_dense_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ CUtensorMap map1,
                      const __grid_constant__ CUtensorMap map2, const __grid_constant__ CUtensorMap map_hi,
@@ -564,7 +564,7 @@ __global__ void __launch_bounds__(kDnThreads, 1)
   const uint32_t half_part = static_cast<uint32_t>(nt) * 64;  // bytes of this CTA's hi (or lo) rows of a stage
   const uint32_t stage_bytes = kWTileBytes + 2 * half_part;
   int tmem_cols = 32;
-  while (tmem_cols < 2 * (nt + p.lo_cols)) tmem_cols <<= 1;
+  while (tmem_cols < (APART ? 4 : 2) * nt) tmem_cols <<= 1;
   const uint32_t acc_stride = static_cast<uint32_t>(tmem_cols) >> 1;
   uint8_t* ring = smem + S::kRing;
 
@@ -674,7 +674,7 @@ __global__ void __launch_bounds__(kDnThreads, 1)
           break;
         }
         tmem_fence_after();
-        const uint32_t d = tmem + static_cast<uint32_t>(b) * acc_stride, dl = d + static_cast<uint32_t>(p.lo_cols);
+        const uint32_t d = tmem + static_cast<uint32_t>(b) * acc_stride, dl = APART ? d + static_cast<uint32_t>(nt) : d;
         for (int ks = 0; ks < k_steps; ++ks) {
           if (!dense_wait_warp(&full[s], ph, p.st)) {
             set_error(p.st, DERR_TIMEOUT);
@@ -683,7 +683,7 @@ __global__ void __launch_bounds__(kDnThreads, 1)
           }
           tmem_fence_after();
           const uint64_t so = static_cast<uint64_t>((s * stage_bytes) >> 4);  // descriptor units of the stage
-          const uint32_t more = ks > 0 ? 1u : 0u, more_lo = p.lo_cols ? more : 1u;
+          const uint32_t more = ks > 0 ? 1u : 0u, more_lo = APART ? more : 1u;
           if (elect_one()) {
 #pragma unroll
             for (int kk = 0; kk < kTileK / 16; ++kk) {
@@ -783,9 +783,9 @@ __global__ void __launch_bounds__(kDnThreads, 1)
       const uint32_t acc = tmem + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(b) * acc_stride;
       auto load_chunk = [&](int col, float (&v)[kDnChunk]) {  // 16 tokens of this thread's weight row
         tmem_ld16(acc + col, v);
-        if (p.lo_cols) {
+        if constexpr (APART) {
           float lo[kDnChunk];
-          tmem_ld16(acc + p.lo_cols + col, lo);
+          tmem_ld16(acc + nt + col, lo);
 #pragma unroll
           for (int i = 0; i < kDnChunk; ++i) v[i] += lo[i];
         }
