@@ -976,7 +976,8 @@ def main() -> None:
             "warmup": args.warmup, "ms_per_step": total_ms / args.steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
             "config": {**workload_config(w), "parallelism": f"replicas x{world}" if world > 1 else "single GPU",
-                       "arithmetic": "fp32 FMA on bf16 weights, fp32 activations and KV cache"},
+                       "arithmetic": "bf16 tensor-core products of bf16 weights with fp32 activations in two bf16 parts (hi + lo), "
+                                     "fp32 accumulation; fp32 KV cache and attention"},
             "e2e": e2e, "gpu_launches": int(args.steps * (pre_l + dec_l)),
             "roofline": roofline, "kernels": kernels, "clocks": clk,
             "prefill_ms": statistics.median(prefill_ms), "decode_ms": dec_ms,

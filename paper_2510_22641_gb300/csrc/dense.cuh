@@ -29,9 +29,10 @@
 //  * The epilogue writes what the next kernel reads -- bf16 parts of q, K, V^T for the attention, of h
 //    for the down projection, of x * gain with the rows' sums of squares for the next normed
 //    projection -- so no launch only converts.
-//  Roles: warp 0 issues TMA (weights before the upstream wait), one thread of the pair's first CTA
-//  issues the MMAs of both, warps 2..9 drain the double-buffered accumulator in two groups of four
-//  (16 tokens at a time, alternating) while the next tile runs.
+//  Roles: warp 0 loads the weights by TMA (from before the upstream wait on), warp 10 the tokens' parts,
+//  warp 1 of the pair's first CTA issues the MMAs of both CTAs, each as a whole warp with one lane
+//  elected; warps 2..9 drain the double-buffered accumulator in two groups of four (16 tokens at a
+//  time, alternating) while the next tile runs.
 #pragma once
 
 #include "gemv.cuh"
