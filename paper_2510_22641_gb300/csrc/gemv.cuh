@@ -626,6 +626,7 @@ __global__ void __launch_bounds__(kGemvThreads, 2)
       const int s = i % kStages;
       if (!mbar_wait(&full[s], static_cast<uint32_t>(i / kStages) & 1u)) {
         set_error(p.st, DERR_TIMEOUT);
+        drain_ring(full, kStages, min(i + kStages, n_units));  // the producer may be done, and past its own check
         break;
       }
       const float* a = reinterpret_cast<const float*>(smem + S::kA + s * S::kActBytes);
