@@ -115,7 +115,8 @@ __device__ __forceinline__ bool mbar_wait_for(uint64_t* bar, uint32_t parity, ui
 }
 
 // The copies of a ring's last fills (stage i % stages, phase i / stages; `issued` in all) may still be landing
-// when a wait gives up: a bounded wait for each before the CTA leaves.
+// when a consumer's wait gives up: a bounded wait for each before the CTA leaves.  The producer waits whether or
+// not a wait has given up, since one may after it is done; it has nothing else to do by then.
 __device__ __forceinline__ void drain_ring(uint64_t* full, int stages, int issued) {
   for (int i = issued > stages ? issued - stages : 0; i < issued; ++i)
     mbar_wait_for(&full[i % stages], static_cast<uint32_t>(i / stages) & 1u, 100000000ull);

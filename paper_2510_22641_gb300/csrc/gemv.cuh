@@ -574,7 +574,7 @@ __global__ void __launch_bounds__(kGemvThreads, 2)
         ph ^= 1;
       }
     }
-    if (lane == 0 && (__ldcg(&p.st->error) & DERR_TIMEOUT)) drain_ring(full, kStages, issued);
+    if (lane == 0) drain_ring(full, kStages, issued);
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer (a whole warp, one lane elected)
     constexpr uint32_t idesc = umma_idesc_bf16(kTileN, 2 * kNPad);
@@ -626,7 +626,6 @@ __global__ void __launch_bounds__(kGemvThreads, 2)
       const int s = i % kStages;
       if (!mbar_wait(&full[s], static_cast<uint32_t>(i / kStages) & 1u)) {
         set_error(p.st, DERR_TIMEOUT);
-        drain_ring(full, kStages, min(i + kStages, n_units));  // the producer may be done, and past its own check
         break;
       }
       const float* a = reinterpret_cast<const float*>(smem + S::kA + s * S::kActBytes);
