@@ -653,8 +653,8 @@ __global__ void __launch_bounds__(kDnThreads, 1)
       }
     }
     // No CTA leaves with a copy in flight, even if a wait gives up only now.  As drain_ring, without its divisions:
-    // stages before s were last filled in this round (parity ph ^ 1), the others in the one before it (or never: that
-    // parity has passed).
+    // stages before s were last filled in the ring's current pass (parity ph ^ 1), the others in the one before it (or
+    // never: that parity has passed).
     if (weights && rank == 0 && lane == 0)
       for (int q = 0; q < stages; ++q) mbar_wait_for(&full[q], q < s ? ph ^ 1 : ph, 100000000ull);
     __syncwarp();
